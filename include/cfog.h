@@ -63,8 +63,8 @@ enum {
     CFOG_CP_EDGE_PEAK = 2,   /* minimum on the border of the search window:
                                 integer offset kept, no sub-pixel refinement    */
     CFOG_CP_FLAT = 3,        /* reserved                                        */
-    CFOG_CP_TIMEOUT = 4      /* a bounded wait of the tensor-core path gave up:
-                                the result is not valid                         */
+    CFOG_CP_TIMEOUT = 4      /* a bounded device-side wait gave up: the result is
+                                not valid                                       */
 };
 
 enum { CFOG_DTYPE_F32 = 0, CFOG_DTYPE_U16 = 1 };
@@ -131,17 +131,17 @@ typedef struct {
     cfog_features sen;
 } cfog_job;
 
-/* Kernel variants of the FFT matcher (threads per CTA / CTAs per SM / FFT plane
- * bound).  0 lets the library choose. */
+/* Kernel variants of the FFT matcher (CTAs of 256 threads per SM / FFT plane
+ * bound).  0 lets the library choose.  Launches with few CPs per SM run CTAs of
+ * 512 threads, one per SM, with the same results. */
 enum {
     CFOG_MATCH_VARIANT_AUTO = 0,
-    CFOG_MATCH_VARIANT_WIDE = 1,   /* 512 threads, 1 CTA per SM, P_y*P_x <= 16384 */
-    CFOG_MATCH_VARIANT_PAIR = 2,   /* 256 threads, 2 CTAs per SM, P_y*P_x <= 9216  */
-    CFOG_MATCH_VARIANT_TRIO = 3,   /* 256 threads, 3 CTAs per SM, P_y*P_x <= 7680,
-                                      spectrum accumulator in tensor memory         */
-    CFOG_MATCH_VARIANT_PAIRT = 4   /* as PAIR, spectrum accumulator in tensor memory
-                                      (TRIO and PAIRT: batched path only; cfog_match
-                                      uses WIDE)                                    */
+    CFOG_MATCH_VARIANT_WIDE = 1,   /* P_y*P_x <= 16384, 2 CTAs per SM (1 above 109 KB of
+                                      shared memory)                                 */
+    CFOG_MATCH_VARIANT_PAIR = 2,   /* P_y*P_x <= 9216, 2 CTAs per SM                 */
+    CFOG_MATCH_VARIANT_TRIO = 3,   /* P_y*P_x <= 7680, 3 CTAs per SM                 */
+    CFOG_MATCH_VARIANT_PAIRT = 4   /* as PAIR, with tuned plans of its own (TRIO and
+                                      PAIRT: batched path only; cfog_match uses WIDE) */
 };
 
 /* Result of one CP (24 bytes).  dx, dy: total integer offset q + v* from the

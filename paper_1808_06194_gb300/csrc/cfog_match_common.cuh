@@ -12,6 +12,7 @@
 
 #include "cfog.h"
 #include "cfog_internal.cuh"
+#include "cfog_plan.cuh"
 
 namespace cfog {
 
@@ -44,6 +45,7 @@ struct MatchArgs {
     int surf_side;   // 2 * radius_max + 1
     int tmpl_max, radius_max;  // launch bounds the shared memory was sized for
     int smem_bytes;  // dynamic shared memory of the launch
+    PlanLimits lim;  // what the FFT matcher's plans may use
     int plan_table;  // tuned-plan table the FFT kernel consults (-1: none)
     long long wait_limit;  // cycle limit of each bounded device-side wait
     int stall_cp;    // failure-detection test: this CP waits on a barrier nothing
@@ -56,13 +58,12 @@ void bf16_test_hook(int *stall_cp, long long *wait_limit);
 
 
 // n / d for 0 <= n < 2^16, 1 <= d < 2^16: one multiply-high with
-// ceil(2^32 / d), exact because n * d < 2^32.
+// ceil(2^32 / d) (which is floor((2^32 - 1) / d) + 1 for d > 1), exact because
+// n * d < 2^32.
 struct FastDiv {
     unsigned mul;
     int d;
-    __device__ explicit FastDiv(int dd) : d(dd) {
-        mul = dd > 1 ? (unsigned)((0x100000000ull + (unsigned)dd - 1) / (unsigned)dd) : 0u;
-    }
+    __device__ explicit FastDiv(int dd) : d(dd) { mul = dd > 1 ? 0xffffffffu / (unsigned)dd + 1u : 0u; }
     __device__ __forceinline__ int div(int n) const { return d > 1 ? (int)__umulhi((unsigned)n, mul) : n; }
 };
 
@@ -237,33 +238,37 @@ __device__ __forceinline__ float block_sum_comp(float v, float2 *red) {
     return r;
 }
 
-// Block-wide compensated sums of K per-thread values at once (the first n are
-// used): the same fixed TwoSum tree as block_sum_comp for each value, with one
-// exchange through shared memory.  out[c] (shared) receives sum c.
-template <int NT, int K>
-__device__ __forceinline__ void block_sum_comp_n(const float *v, int n, float2 (*red)[NT / 32],
+// Block-wide compensated sums of K values at once (the first n are used) over
+// VT partial sums, VT / NT per thread (v[h]: partial sum tid + h * NT) of the
+// first NT threads: the same fixed TwoSum tree as block_sum_comp of VT threads for each value, with
+// one exchange through shared memory.  out[c] (shared) receives sum c.
+template <int VT, int NT, int K>
+__device__ __forceinline__ void block_sum_comp_n(const float (*v)[K], int n, float2 (*red)[VT / 32],
                                                  float *out) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
-    for (int c = 0; c < K; ++c) {
-        if (c >= n) break;
-        float hi = v[c], lo = 0.f;
+    for (int h = 0; h < VT / NT && threadIdx.x < NT; ++h) {
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            const float oh = __shfl_xor_sync(0xffffffffu, hi, o);
-            const float ol = __shfl_xor_sync(0xffffffffu, lo, o);
-            float sum, err;
-            two_sum(hi, oh, sum, err);
-            hi = sum;
-            lo = (lo + ol) + err;
+        for (int c = 0; c < K; ++c) {
+            if (c >= n) break;
+            float hi = v[h][c], lo = 0.f;
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                const float oh = __shfl_xor_sync(0xffffffffu, hi, o);
+                const float ol = __shfl_xor_sync(0xffffffffu, lo, o);
+                float sum, err;
+                two_sum(hi, oh, sum, err);
+                hi = sum;
+                lo = (lo + ol) + err;
+            }
+            if (lane == 0) red[c][warp + h * (NT / 32)] = make_float2(hi, lo);
         }
-        if (lane == 0) red[c][warp] = make_float2(hi, lo);
     }
     __syncthreads();
     if (threadIdx.x < n) {
         const int c = threadIdx.x;
         float h = red[c][0].x, l = red[c][0].y;
-        for (int w = 1; w < NT / 32; ++w) {
+        for (int w = 1; w < VT / 32; ++w) {
             float sum, err;
             two_sum(h, red[c][w].x, sum, err);
             h = sum;
@@ -272,6 +277,31 @@ __device__ __forceinline__ void block_sum_comp_n(const float *v, int n, float2 (
         out[c] = h + l;
     }
 }
+
+// The FFT matcher's geometry (cfog_match_fft.cuh): threads per CTA, and the
+// tensor-memory columns of a CTA (512 per SM, a power of two) that hold the
+// spectrum accumulators.
+constexpr int kFftThreads = 256;
+constexpr int kMaxRadius = 32;
+constexpr int kPlanTables = 2;
+constexpr int fft_tmem_cols(int per_sm) { return per_sm >= 3 ? 128 : 256; }
+constexpr int kFftThreadsTall = 512;   // CTAs of launches that leave an SM one CP
+
+// The FFT matcher's kernel of one geometry (one translation unit each): its
+// launch, and the write of n tuned-plan entries of one of its tables on the
+// current device.
+struct MatchKernel {
+    const void *fn;
+    int threads, tmem_cols;
+    cfog_status (*launch)(const MatchArgs &a, int *counter, const int *order, int grid, int smem,
+                          cudaStream_t s);
+    cfog_status (*write_plans)(int table, size_t offset, const int32_t *src, size_t n);
+};
+MatchKernel match_kernel_wide();
+MatchKernel match_kernel_pair();
+MatchKernel match_kernel_trio();
+MatchKernel match_kernel_wide_tall();
+MatchKernel match_kernel_pair_tall();
 
 // Launch the BF16 direct-correlation matcher (cfog_bf16.cu): one CTA per CP
 // when `order` is null, otherwise persistent CTAs draining the queue.

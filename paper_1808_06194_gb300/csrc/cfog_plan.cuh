@@ -9,9 +9,9 @@
 // with P >= b + 2r gives every lag in [-r, r] without circular wrap.  Every
 // FFT length is a product P = A * B of two register radices, A, B in
 // {2,3,4,5,6,8,9,10,12,15,16} (B = 1 allowed): two shared-memory passes per
-// axis.  The plan depends only on (N, r, m) and the kernel variant's plane
-// bound, so a CP's result never depends on its batch.  The search is exact
-// integer arithmetic: host and device agree.
+// axis.  The plan depends only on (N, r, m) and the kernel variant's limits,
+// so a CP's result never depends on its batch.  The search is exact integer
+// arithmetic: host and device agree.
 #pragma once
 
 #include <cstdint>
@@ -22,17 +22,21 @@ constexpr int kMaxFft = 256;           // longest supported FFT side
 constexpr int kMaxPlaneElems = 16384;  // largest P_y * P_x of any kernel variant
 constexpr int kNbMax = 4;              // blocks per axis searched
 constexpr int kPTries = 4;             // FFT lengths tried per axis
+constexpr int kMaxPlanes = 4;          // planes transformed side by side
+constexpr int kBoxRows = 4;            // window rows a warp takes at a time in the box sums
 
 struct FftDim {
     int nb;   // number of template blocks along this axis
     int bs;   // block size ceil(N / nb); the last block may be shorter
     int P;    // FFT length, even
-    int A;    // stage-1 radix (stride B)
+    int A;    // stage-1 radix (stride B), A >= B
     int B;    // stage-2 radix (contiguous); 1 = single stage
 };
 
 struct MatchPlan {
     FftDim y, x;
+    int ld;   // row pitch of a plane, in complex values (odd)
+    int G;    // planes transformed side by side: (block, channel) items per round
 };
 
 constexpr bool is_radix(int R) {
@@ -41,9 +45,10 @@ constexpr bool is_radix(int R) {
 }
 
 // Split of every even length P <= kMaxFft into A * B (register radices, B may
-// be 1), as balanced as possible (ties: smaller A), and the smallest
-// splittable length >= P.  Built at compile time; the host and the device
-// read the same table.
+// be 1, A >= B), as balanced as possible, and the smallest splittable length
+// >= P.  The larger radix comes first: the last column pass holds two
+// butterflies of radix B and their accumulators in registers.  Built at
+// compile time; the host and the device read the same table.
 struct SmoothTable {
     unsigned char A[kMaxFft + 1];
     unsigned char B[kMaxFft + 1];
@@ -57,8 +62,8 @@ struct SmoothTable {
             for (int a = 2; a <= 16; ++a) {
                 if (!is_radix(a) || P % a) continue;
                 const int b = P / a;
-                if (b != 1 && !is_radix(b)) continue;
-                const int d = a > b ? a - b : b - a;
+                if (b > a || (b != 1 && !is_radix(b))) continue;
+                const int d = a - b;
                 if (d < bestd) {
                     bestd = d;
                     bestA = a;
@@ -84,19 +89,57 @@ __host__ __device__ inline const SmoothTable &smooth_table() {
 #endif
 }
 
-// Split an even P into A * B; returns false when no split exists.
-__host__ __device__ inline bool fft_split(int P, int *A, int *B) {
-    const SmoothTable &t = smooth_table();
-    if (P < 0 || P > kMaxFft || !t.A[P]) return false;
-    *A = t.A[P];
-    *B = t.B[P];
-    return true;
-}
-
 __host__ __device__ inline int ceil_log2(int v) {
     int c = 0;
     while ((1 << c) < v) ++c;
     return c;
+}
+
+// What a kernel variant gives a plan.
+struct PlanLimits {
+    int maxe;       // bound of P_y * P_x
+    int smem_cap;   // dynamic shared memory of one CTA at the variant's CTAs per SM
+    int tm_cols;    // tensor-memory columns per thread for the accumulators
+    int threads;    // threads per CTA
+};
+
+// Floats of a staged row of raw pixels for an FFT of Px columns: 16-byte
+// copies start at the 4-pixel boundary at or before its first column.
+__host__ __device__ inline int raw_len(int Px) { return (Px + 3 + 3) & ~3; }
+
+// Row pitch of a plane in complex values: odd, so that threads walking down a
+// column of complex values hit distinct banks, and wide enough that a row's
+// raw window and template pixels (from a 16-byte boundary of the row) fit into
+// the row they are transformed in.
+__host__ __device__ inline int plane_pitch(int Px) { return raw_len(Px) + 1; }
+
+// Floats per plane (a multiple of 4: every plane starts on a 16-byte boundary).
+__host__ __device__ inline int plane_floats(int Py, int ld) { return (2 * Py * ld + 3) & ~3; }
+
+// Scratch floats of the box sums: row sums at an odd pitch and kBoxRows prefix rows per warp.
+__host__ __device__ inline int box_floats(int N, int r, int threads) {
+    const int W = N + 2 * r, L = 2 * r + 1;
+    return W * (L | 1) + (threads / 32) * kBoxRows * (W + 1);
+}
+
+// Tensor-memory columns one thread needs for the accumulators: 2 B floats of
+// every column butterfly pair it owns, in chunks of 16 columns.
+__host__ __device__ inline int accum_chunk(int By) { return By <= 8 ? 16 : 32; }
+__host__ __device__ inline int accum_cols(const FftDim &y, const FftDim &x, int threads) {
+    const int pairs = y.A * (x.P / 2 + 1);
+    return (pairs + threads - 1) / threads * accum_chunk(y.B);
+}
+
+// Floats before the twiddles: n planes, or the box-sum scratch.
+__host__ __device__ inline int plan_region(const MatchPlan &p, int N, int r, int threads, int n) {
+    const int planes = n * plane_floats(p.y.P, p.ld), box = (box_floats(N, r, threads) + 1) & ~1;
+    return planes > box ? planes : box;
+}
+
+// Dynamic shared memory of the FFT matcher for a plan with n planes: the planes,
+// the twiddles of both axes and the (2r+1)^2 scores.
+__host__ __device__ inline int plan_smem_bytes(const MatchPlan &p, int N, int r, int threads, int n) {
+    return 4 * (plan_region(p, N, r, threads, n) + 2 * (p.y.P + p.x.P) + (2 * r + 1) * (2 * r + 1));
 }
 
 // Integer cost of one length-P pass over a plane: each stage is a
@@ -105,51 +148,18 @@ __host__ __device__ inline int fft_len_cost(int A, int B) {
     return 100 + 12 * ceil_log2(A) + (B > 1 ? 100 + 12 * ceil_log2(B) : 0);
 }
 
-// Best (Py, Px) for one block split (nby, nbx) with P_y * P_x <= maxe (the
-// kernel variant's shared-memory plane); returns the cost (or -1 when no
-// size fits) and fills *out.  Scan order: Py ascending, then Px ascending;
-// a later candidate wins only with a strictly smaller cost.
-__host__ __device__ inline long long plan_for_split(int N, int r, int m, int nby, int nbx,
-                                                    int maxe, MatchPlan *out) {
-    const int bsy = (N + nby - 1) / nby, bsx = (N + nbx - 1) / nbx;
-    if ((nby - 1) * bsy >= N || (nbx - 1) * bsx >= N) return -1;
-    const int needy = bsy + 2 * r, needx = bsx + 2 * r;
-    long long best = -1;
-    if (needy > kMaxFft || needx > kMaxFft) return -1;
-    const SmoothTable &t = smooth_table();
-    int tried_y = 0;
-    for (int Py = t.next[needy]; Py != 0 && tried_y < kPTries; Py = t.next[Py + 1]) {
-        const int Ay = t.A[Py], By = t.B[Py];
-        ++tried_y;
-        int tried_x = 0;
-        for (int Px = t.next[needx]; Px != 0 && tried_x < kPTries; Px = t.next[Px + 1]) {
-            const int Ax = t.A[Px], Bx = t.B[Px];
-            ++tried_x;
-            if (Py * Px > maxe) continue;
-            // the row box sums of the ||D||^2 window (W x L floats) use the plane
-            // as scratch before the FFTs
-            if (2LL * Py * (Px + 1) < (long long)(N + 2 * r) * (2 * r + 1)) continue;
-            const long long per = (long long)Py * Px * (fft_len_cost(Ay, By) + fft_len_cost(Ax, Bx));
-            const long long cost = per * (long long)(nby * nbx * m + 1);
-            if (best < 0 || cost < best) {
-                best = cost;
-                out->y = FftDim{nby, bsy, Py, Ay, By};
-                out->x = FftDim{nbx, bsx, Px, Ax, Bx};
-            }
-        }
-    }
-    return best;
-}
-
 // A plan named by a code: bits 4..7 the split index l (nby = l / kNbMax + 1,
 // nbx = l % kNbMax + 1), bits 2..3 and 0..1 which of the first kPTries
-// splittable lengths >= b + 2r the y and x axes take.  Returns the cost of
-// plan_for_split's model (or -1 when the code names no feasible plan) and
-// fills *out.  The autotuner times codes and records the fastest per class.
+// splittable lengths >= b + 2r the y and x axes take.  Returns its cost (or
+// -1 when the code names no feasible plan) and fills *out.  The cost model's
+// plan is the code of least cost, ties to the smaller code; the autotuner
+// times codes and records the fastest per class.  A plane that leaves room
+// for one CTA per SM only costs twice as much: it makes every CP of the launch
+// run that way.
 constexpr int kPlanCodes = kNbMax * kNbMax * kPTries * kPTries;
 
-__host__ __device__ inline long long plan_for_code(int N, int r, int m, int code, int maxe,
-                                                   MatchPlan *out) {
+__host__ __device__ inline long long plan_for_code(int N, int r, int m, int code,
+                                                   const PlanLimits &lim, MatchPlan *out) {
     if (code < 0 || code >= kPlanCodes) return -1;
     const int l = code >> 4, ty = (code >> 2) & 3, tx = code & 3;
     const int nby = l / kNbMax + 1, nbx = l % kNbMax + 1;
@@ -162,40 +172,40 @@ __host__ __device__ inline long long plan_for_code(int N, int r, int m, int code
     for (int i = 0; i < ty && Py != 0; ++i) Py = t.next[Py + 1];
     int Px = t.next[needx];
     for (int i = 0; i < tx && Px != 0; ++i) Px = t.next[Px + 1];
-    if (Py == 0 || Px == 0 || Py * Px > maxe) return -1;
-    if (2LL * Py * (Px + 1) < (long long)(N + 2 * r) * (2 * r + 1)) return -1;
+    if (Py == 0 || Px == 0 || Py * Px > lim.maxe) return -1;
     const int Ay = t.A[Py], By = t.B[Py], Ax = t.A[Px], Bx = t.B[Px];
-    const long long per = (long long)Py * Px * (fft_len_cost(Ay, By) + fft_len_cost(Ax, Bx));
     out->y = FftDim{nby, bsy, Py, Ay, By};
     out->x = FftDim{nbx, bsx, Px, Ax, Bx};
-    return per * (long long)(nby * nbx * m + 1);
+    if (accum_cols(out->y, out->x, lim.threads) > lim.tm_cols) return -1;
+    out->ld = plane_pitch(Px);
+    out->G = 1;
+    const int items = nby * nbx * m;
+    const int fixed = plan_smem_bytes(*out, N, r, lim.threads, 1);
+    const int plane = 4 * plane_floats(Py, out->ld);
+    if (fixed <= lim.smem_cap) {
+        // as many planes as fit, spread evenly over the rounds
+        const int room = (lim.smem_cap - 4 * (2 * (Py + Px) + (2 * r + 1) * (2 * r + 1))) / plane;
+        int g = room < items ? room : items;
+        g = g < kMaxPlanes ? g : kMaxPlanes;
+        const int rounds = (items + g - 1) / g;
+        out->G = (items + rounds - 1) / rounds;
+    }
+    const long long per = (long long)Py * Px * (fft_len_cost(Ay, By) + fft_len_cost(Ax, Bx));
+    const long long cost = per * (long long)(items + 1);
+    return fixed <= lim.smem_cap ? cost : 2 * cost;
 }
 
-// Split index l in [0, kNbMax^2): nby = l / kNbMax + 1, nbx = l % kNbMax + 1.
-// The plan is the split with the smallest cost, ties to the smaller l.
-__host__ inline bool make_plan_host(int N, int r, int m, int maxe, MatchPlan *out) {
+__host__ inline bool make_plan_host(int N, int r, int m, const PlanLimits &lim, MatchPlan *out) {
     long long best = -1;
-    for (int l = 0; l < kNbMax * kNbMax; ++l) {
+    for (int code = 0; code < kPlanCodes; ++code) {
         MatchPlan p;
-        const long long c = plan_for_split(N, r, m, l / kNbMax + 1, l % kNbMax + 1, maxe, &p);
+        const long long c = plan_for_code(N, r, m, code, lim, &p);
         if (c >= 0 && (best < 0 || c < best)) {
             best = c;
             *out = p;
         }
     }
     return best >= 0;
-}
-
-// Row pitch of the shared-memory plane: odd, so that threads walking down a
-// column of complex values hit distinct banks.
-__host__ __device__ inline int plane_ld(const MatchPlan &p) { return p.x.P + 1; }
-
-// Dynamic shared memory of the FP32 FFT match kernel for a plan and radius r:
-// the complex plane, the twiddles of both axes, the accumulator position
-// table and the (2r+1)^2 box sums.
-__host__ __device__ inline int plan_smem_bytes(const MatchPlan &p, int r) {
-    return p.y.P * plane_ld(p) * 8 + (p.y.P + p.x.P) * 8 + p.y.P * (p.x.P / 2 + 1) * 4 +
-           (2 * r + 1) * (2 * r + 1) * 4;
 }
 
 }  // namespace cfog
