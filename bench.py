@@ -39,13 +39,11 @@ RMIN, RMAX = 8, 20
 MARGIN = 64 + RMAX + 16   # half template + radius + largest true offset
 SEED_PAIR = 1
 SEED_CP = 101
-# DRAM read + write bytes per CP of the batched matcher (pair-TMEM variant, the
-# autotuner's pick on GB300), from an ncu capture of 144 CPs of this workload
-# (dram__bytes_read.sum + dram__bytes_write.sum = 128.74 MB + 3.26 MB).  Set to
-# None when the kernel changes.
-MATCH_TRAFFIC_PER_CP = 132.01e6 / 144
-MATCH_TRAFFIC_NOTE = ("DRAM bytes of one ncu capture of 144 CPs (132.0 MB, pair-TMEM variant) "
-                      "scaled to this launch by CP count")
+# DRAM read + write bytes per CP of the batched matcher, from an ncu capture of
+# 1024 CPs of this workload (dram__bytes_read.sum + dram__bytes_write.sum =
+# 1125.34 MB + 17.23 MB).  Set to None when the kernel changes.
+MATCH_TRAFFIC_PER_CP = 1142.57e6 / 1024
+MATCH_TRAFFIC_NOTE = "DRAM bytes of one ncu capture of a 1024-CP launch (1142.6 MB), scaled by CP count"
 E2E_PIPE_STEPS = 40   # timed steps per pipelined end-to-end run (three runs, median)
 WORKLOAD = "batched 2048x2048 f32 pair, 1024 Harris CPs (32x32 grid), N in {48,64,96,128}, r in 8..20"
 
@@ -569,7 +567,7 @@ def bench_ours(args):
                     "frac": achieved / hbm_peak, "peak_note": hbm_note,
                     "traffic": MATCH_TRAFFIC_PER_CP * n if (full and MATCH_TRAFFIC_PER_CP) else None,
                     "traffic_note": MATCH_TRAFFIC_NOTE,
-                    "kernel": "match_persistent_kernel",
+                    "kernel": "match_fft_kernel",
                     "bytes_per_launch": gbytes,
                     "unique_bytes_per_launch": match_unique_bytes(args.size),
                     "bytes_rule": "4 m (N^2 + W^2) per CP, W = N + 2r, m = 9"}
