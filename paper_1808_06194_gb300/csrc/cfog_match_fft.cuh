@@ -375,9 +375,11 @@ __device__ __forceinline__ void col_s2_accumulate(const float *planes, int pf, i
 
 // Inverse column pass 2 from the accumulators: the Hermitian pair of every
 // butterfly is formed in registers, transformed and written to the plane.
+// Frequency 0 goes to *dc instead: it adds the same to every lag, most of C,
+// and the inverse of the rest rounds at the size of the rest.
 template <int NT, int Bv>
 __device__ __noinline__ void col_inv_s2(float2 *plane, int ld, int Ay, FastDiv divH,
-                                        const unsigned *cols, uint32_t tm) {
+                                        const unsigned *cols, uint32_t tm, float *dc) {
     constexpr int CH = Bv <= 8 ? 16 : 32;
     const int Hx = divH.d;
     const int total = Ay * Hx;
@@ -386,6 +388,10 @@ __device__ __noinline__ void col_inv_s2(float2 *plane, int ld, int Ay, FastDiv d
         float acc[CH];
 #pragma unroll
         for (int c = 0; c < CH; c += 16) tmem_ld16(tm + c, acc + c);
+        if (it == 0) {
+            *dc = acc[0];
+            acc[0] = 0.f;
+        }
         const bool ok = it < total;
         const int a = ok ? divH.div(it) : 0;
         const unsigned pk = ok ? cols[it - a * Hx] : 0u;
@@ -443,8 +449,9 @@ __device__ __noinline__ void col_inv_s1(float2 *plane, int ld, const float2 *tw,
 // Inverse row pass 1 over the L rows of lags, j fastest, fused with the
 // assembly of Eq. 5: surf holds the window energy's deviation from N^2 (box
 // sums of ||D_sen||^2 - 1) and receives S = (sum T^2 + N^2) - 2 C + deviation;
-// the product with the (two-part) scale is added to the high part in one
-// rounding.
+// base holds (sum T^2 + N^2) - 2 C's share of frequency 0, as an exact two-part
+// sum, and the product with the (two-part) scale is added to its high part in
+// one rounding.
 template <int NT, int A>
 __device__ __noinline__ void row_inv_s1(const float2 *plane, int ld, const float2 *tw, FastDiv divB,
                                         int L, float2 scale, float2 base, float *surf) {
@@ -615,7 +622,8 @@ struct CoreShared {
     Item item[2][V::NT > kFftThreads ? 2 * kMaxPlanes : kMaxPlanes]; // this round's items and the next one's
     CpView cv;                // the CP and its plan: kept here, not in registers, so that
     MatchPlan plan;           // the passes have the register file to themselves
-    float dc_err;             // rounding error of the accumulated frequency 0
+    float dc;                 // accumulated frequency 0 ...
+    float dc_err;             // ... and what its sum rounded off
     float zero[kMaxFft];      // a row of zeros
 };
 
@@ -816,8 +824,10 @@ __device__ __forceinline__ void match_one(const MatchArgs &A, const int cp, Core
     }
 
     // the inverse passes backwards, then S(v) in surf
-    const float tt = (float)block_sum<NT>(tt_part, sh.red_l) * (1.0f / kEnergyScale);
-    CFOG_RADIX_SWITCH1(DY.B, (col_inv_s2<NT, RR>(plane0, ld, DY.A, divH, sh.cols, tm)));
+    const auto tt_sum = block_sum<NT>(tt_part, sh.red_l);
+    const float tt_hi = (float)tt_sum;
+    const float tt = tt_hi * (1.0f / kEnergyScale);
+    CFOG_RADIX_SWITCH1(DY.B, (col_inv_s2<NT, RR>(plane0, ld, DY.A, divH, sh.cols, tm, &sh.dc)));
     __syncthreads();
     CFOG_RADIX_SWITCH(DY.A, (col_inv_s1<NT, RR>(plane0, ld, twy, DY.B, divP, Lside)));
     __syncthreads();
@@ -831,8 +841,12 @@ __device__ __forceinline__ void match_one(const MatchArgs &A, const int cp, Core
         float2 scale, base;
         scale.x = -0.5f / area;
         scale.y = fmaf(-scale.x, area, -0.5f) / area;
-        two_sum(tt, (float)N * (float)N, base.x, base.y);
-        base.y = fmaf(sh.dc_err, scale.x, base.y);
+        const float dc = sh.dc, c0 = dc * scale.x;
+        float e1, e2, energy;
+        two_sum(tt, (float)N * (float)N, energy, e1);
+        two_sum(energy, c0, base.x, e2);
+        base.y = e1 + e2 + fmaf(dc, scale.x, -c0) + fmaf(dc, scale.y, sh.dc_err * scale.x) +
+                 (float)(tt_sum - (decltype(tt_sum))tt_hi) * (1.0f / kEnergyScale);
         CFOG_RADIX_SWITCH(DX.A, (row_inv_s1<NT, RR>(plane0, ld, twx, divBx, Lside, scale, base, surf)));
     }
     __syncthreads();
