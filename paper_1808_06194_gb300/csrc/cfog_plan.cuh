@@ -155,7 +155,12 @@ __host__ __device__ inline int fft_len_cost(int A, int B) {
 // plan is the code of least cost, ties to the smaller code; the autotuner
 // times codes and records the fastest per class.  A plane that leaves room
 // for one CTA per SM only costs twice as much: it makes every CP of the launch
-// run that way.
+// run that way.  Of the 16384-element planes it costs a quarter more from
+// radius kWideRadius on: there a block's window is mostly margin, and small
+// blocks transform up to twice the elements (1000 CPs of N 128, a quarter more
+// against double: r 32 3.0 and 5.3 ms, r 28 2.9 and 3.5, r 24 3.0 and 2.5; 49 CPs:
+// r 28 0.48 and 0.66, r 24 the same).
+constexpr int kWideRadius = 26;
 constexpr int kPlanCodes = kNbMax * kNbMax * kPTries * kPTries;
 
 __host__ __device__ inline long long plan_for_code(int N, int r, int m, int code,
@@ -192,7 +197,8 @@ __host__ __device__ inline long long plan_for_code(int N, int r, int m, int code
     }
     const long long per = (long long)Py * Px * (fft_len_cost(Ay, By) + fft_len_cost(Ax, Bx));
     const long long cost = per * (long long)(items + 1);
-    return fixed <= lim.smem_cap ? cost : 2 * cost;
+    if (fixed <= lim.smem_cap) return cost;
+    return r >= kWideRadius && lim.maxe == kMaxPlaneElems ? cost + cost / 4 : 2 * cost;
 }
 
 __host__ inline bool make_plan_host(int N, int r, int m, const PlanLimits &lim, MatchPlan *out) {
