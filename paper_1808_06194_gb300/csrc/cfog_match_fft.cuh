@@ -142,12 +142,12 @@ __device__ __forceinline__ void stage_rows(float2 *plane, int ld, int off, const
     const uint32_t dstep = (uint32_t)(NW * ld * 8);   // NW is even: the raw rows' offset stays
     const int64_t sstep = rp * NW;
     for (int x = lane * F; x < len; x += 32 * F) {
-        const int valid = F == 4 ? 4 * min(max(x1 - x, 0), 4) : (x >= x0 && x < x1 ? 4 : 0);
+        const StageCopy c = stage_copy(F, x, x0, x1);
         uint32_t dst = smem_u32(raw_row(plane, ld, warp) + off + x);
-        const float *s = src + warp * rp + (valid ? x : x0);
+        const float *s = src + warp * rp + c.col;
 #pragma unroll 4
         for (int y = warp; y < rows; y += NW) {
-            cp_async_fill<BYTES>(dst, s, valid);
+            cp_async_fill<BYTES>(dst, s, c.bytes);
             dst += dstep;
             s += sstep;
         }

@@ -107,6 +107,23 @@ struct PlanLimits {
 // copies start at the 4-pixel boundary at or before its first column.
 __host__ __device__ inline int raw_len(int Px) { return (Px + 3 + 3) & ~3; }
 
+// Where a staging copy of F floats (4: 16 bytes, 1: 4 bytes) for column x of a
+// raw row takes its bytes: a lane copies columns [x, x + F) behind the 4-pixel
+// boundary, of which those in [x0, x1) are wanted.
+struct StageCopy {
+    int col;     // first source column behind the boundary
+    int bytes;   // bytes read from there; the rest of the copy becomes zero
+};
+__host__ __device__ inline StageCopy stage_copy(int F, int x, int x0, int x1) {
+    if (F == 4) {
+        const int n = x1 - x < 4 ? x1 - x : 4;
+        // a copy that reads nothing still names an address, which has to be
+        // aligned to the copy's size and inside the row: the boundary itself
+        return n > 0 ? StageCopy{x, 4 * n} : StageCopy{0, 0};
+    }
+    return x >= x0 && x < x1 ? StageCopy{x, 4} : StageCopy{x0, 0};
+}
+
 // Row pitch of a plane in complex values: odd, so that threads walking down a
 // column of complex values hit distinct banks, and wide enough that a row's
 // raw window and template pixels (from a 16-byte boundary of the row) fit into
