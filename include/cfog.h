@@ -63,8 +63,11 @@ enum {
     CFOG_CP_EDGE_PEAK = 2,   /* minimum on the border of the search window:
                                 integer offset kept, no sub-pixel refinement    */
     CFOG_CP_FLAT = 3,        /* reserved                                        */
-    CFOG_CP_TIMEOUT = 4      /* a bounded device-side wait gave up: the result is
+    CFOG_CP_TIMEOUT = 4,     /* a bounded device-side wait gave up: the result is
                                 not valid                                       */
+    CFOG_CP_NONFINITE = 5    /* no lag has a finite score (NaN or infinite pixels in
+                                the template or window): no match, the prior kept,
+                                ssd infinite                                    */
 };
 
 enum { CFOG_DTYPE_F32 = 0, CFOG_DTYPE_U16 = 1 };

@@ -774,8 +774,21 @@ __device__ void match_one_bf16(const MatchArgs &A, const int cp, Bf16Shared &sh,
         float smin;
         int imin;
         block_argmin<BT>(bv, bi, sh.red_f, sh.red_i, smin, imin);
-        if (t == 0) s0 = smin;
-        if (t > 0 && !(smin <= s0 + band)) break;   // uniform: every thread has smin
+        // uniform: every thread has smin and imin
+        if (t == 0) {
+            s0 = smin;
+            if (!isfinite(smin)) {
+                // NaN or infinite features leave no lag to choose (imin may be no lag at all)
+                if (tid == 0) {
+                    res.status = CFOG_CP_NONFINITE;
+                    A.out[cp] = res;
+                }
+                __syncthreads();
+                return;
+            }
+        } else if (imin == INT_MAX || !(smin <= s0 + band)) {
+            break;
+        }
         if (tid == 0) {
             sh.cand_idx[t] = imin;
             sh.ncand = t + 1;

@@ -864,12 +864,14 @@ __device__ __forceinline__ void match_one(const MatchArgs &A, const int cp, Core
     float smin;
     int imin;
     block_argmin<NT>(bv, bi, sh.red_f, sh.red_i, smin, imin);
+    // NaN or infinite features leave no lag to choose (imin may be no lag at all)
+    const bool found = isfinite(smin);
 
     // lags inside the nomination band are re-scored directly
     const float band = kRescoreRel * (tt + (float)N * (float)N);
     for (int i = tid; i < L2; i += NT) {
         const float sv = surf[i];
-        if (sv <= smin + band) {
+        if (found && sv <= smin + band) {
             const int slot = atomicAdd(&sh.cand_n, 1);
             if (slot < kCandBuf) {
                 sh.cand_idx[slot] = i;
@@ -1013,7 +1015,10 @@ __device__ __forceinline__ void match_one(const MatchArgs &A, const int cp, Core
         }
     }
 
-    if (tid == 0) {
+    if (tid == 0 && !found) {
+        res.status = CFOG_CP_NONFINITE;
+        A.out[cp] = res;
+    } else if (tid == 0) {
         const int vy = win / Lside - r, vx = win - (win / Lside) * Lside - r;
         res.dx = qx + vx;
         res.dy = qy + vy;
