@@ -880,8 +880,29 @@ __device__ __forceinline__ void match_one(const MatchArgs &A, const int cp, Core
         }
     }
     __syncthreads();
-    int ncand = min(sh.cand_n, kCandBuf);
-    if (tid == 0) {
+    int ncand = sh.cand_n;
+    if (ncand > kCandBuf) {
+        // more lags than the buffer holds (a flat or periodic window), and which of
+        // them entered it depends on timing: the best kMaxCand by (FFT value, index)
+        // are picked from the surface, one arg-min behind the last at a time
+        float pv = smin;
+        int pi = imin;
+        if (tid == 0) sh.cand_idx[0] = imin;
+        for (int c = 1; c < kMaxCand; ++c) {
+            float v = INFINITY;
+            int at = INT_MAX;
+            for (int i = tid; i < L2; i += NT) {
+                const float sv = surf[i];
+                if ((sv > pv || (sv == pv && i > pi)) && (sv < v || (sv == v && i < at))) {
+                    v = sv;
+                    at = i;
+                }
+            }
+            block_argmin<NT>(v, at, sh.red_f, sh.red_i, pv, pi);
+            if (tid == 0) sh.cand_idx[c] = pi;
+        }
+        ncand = kMaxCand;
+    } else if (tid == 0) {
         // order by (FFT value, index) and keep the best kMaxCand
         for (int a = 1; a < ncand; ++a) {
             const int ii = sh.cand_idx[a];
