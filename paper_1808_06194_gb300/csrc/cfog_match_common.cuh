@@ -16,7 +16,7 @@
 
 namespace cfog {
 
-constexpr float kRescoreRel = 2e-5f; // FFT nomination band, relative to sum T^2 + N^2
+constexpr float kRescoreRel = 2e-5f; // FFT nomination band, relative to the energies of template and window
 constexpr int kMaxCand = 8;
 constexpr int kCandBuf = 64;
 

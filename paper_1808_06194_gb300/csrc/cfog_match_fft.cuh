@@ -9,14 +9,14 @@
 // the sum over channels of the 2-D correlations, so the channel FFT is not
 // needed.  Per channel k the template block (real part) and its window
 // (imaginary part) share one complex 2-D FFT; the two spectra are separated
-// by Hermitian symmetry and conj(T_k) S_k is accumulated with weight -2; one
-// inverse 2-D FFT then yields -2 C(v) at every lag.  The box sums of
-// ||D_sen||^2 (the middle term of Eq. 5) come from two separable sliding-sum
-// passes before the FFTs, and S(v) = sum T^2 + B(v) - 2 C(v).
-// The FFT surface nominates the minimum; lags within a relative 2e-5 of it
-// are re-scored directly (FP32 differences and sums, compensated block
-// reduction), so the argmin is decided at the precision of the features.  The quadratic sub-pixel fit runs
-// in FP64 on the 3 x 3 neighbourhood.
+// by Hermitian symmetry, and conj(T_k) S_k is accumulated (with a factor 4, taken
+// out together with the -2 at the end); one inverse 2-D FFT then yields C(v) at
+// every lag.  The middle term of Eq. 5 comes before the FFTs, from sums of
+// ||D_sen||^2 - pivot: prefix sums of the rows, sliding sums down the columns.
+// The FFT surface nominates the minimum; lags within 2e-5 of the energies behind
+// it are re-scored directly (FP32 differences and sums, compensated block
+// reduction), so the argmin is decided at the precision of the features.  The
+// quadratic sub-pixel fit runs in FP64 on the 3 x 3 neighbourhood.
 //
 // Each FFT length is P = A * B: a decimation-in-frequency pass of radix A at
 // stride B (then twiddles) and a pass of radix B on contiguous runs, each a
@@ -86,6 +86,8 @@ struct CpView {
     JobView J;
     int ry0, rx0, sy0, sx0;   // template origin (reference), window origin (sensed)
     int N, r, m;
+    float pivot;              // of the window's energy (box_sums)
+    float scale;              // of the template's (row_fwd_s1)
 };
 
 // One (block, channel) item: where its window and template pixels lie.
@@ -182,10 +184,15 @@ __device__ __forceinline__ void stage_items(const Item *items, int64_t srp, int6
     X(90, 10, 9) X(96, 12, 8) X(100, 10, 10) X(108, 12, 9) X(120, 12, 10) X(128, 16, 8)           \
     X(144, 12, 12) X(160, 16, 10) X(180, 15, 12)
 
-// Fixed-point scale of sum T^2: a lane's share of a row is at most 16 (CFOG
-// vectors have unit norm) and a float's digits fit exactly, the CP's sum at
-// most 2^16.
-constexpr float kEnergyScale = 4294967296.f;
+// sum T^2 is a sum of integers, which does not depend on which thread took which
+// row: lanes' shares of a row times a power of two that brings the CP's sum, as a
+// sample of the template estimates it, to 2^38 or twice that.  From 2^32 on the
+// shares' rounding is below a float's, and up to 2^20 shares of at most 2^42 add
+// up.  A sum outside [2^32, 2^42) (the sample saw a part of the template that is
+// far from the rest) is taken again by energy_direct.
+constexpr int kEnergyExp = 38;
+constexpr long long kEnergyMin = 1LL << 32;
+constexpr float kEnergyMax = 4398046511104.f;      // 2^42
 
 // Row pass 1 (radix A at stride B) on one plane, reading the raw pixels in
 // place: template + i window.  A warp takes whole rows (32 / B of them, B
@@ -196,12 +203,11 @@ constexpr float kEnergyScale = 4294967296.f;
 // half of all shared-memory wavefronts were conflicts).  Rows outside the
 // window or the template read `zero`; rows from the window's height up to Py
 // are written as zeros.  BC: B if known at compile time, else 0.  Returns the
-// lane's share of sum T^2, in fixed point: integer sums do not depend on which
-// thread took which row.
+// lane's share of sum T^2 times `scale`.
 template <int NT, int A, int BC>
 __device__ __forceinline__ long long row_fwd_s1(float2 *plane, int ld, const float2 *tw, FastDiv divB,
                                             int D, int Py, int len, const Item &q, const float *zero,
-                                            int warp0) {
+                                            int warp0, float scale) {
     const int lane = threadIdx.x & 31;
     const int B = BC ? BC : divB.d;
     const int R = BC ? 32 / (BC ? BC : 1) : divB.div(32);
@@ -246,7 +252,7 @@ __device__ __forceinline__ long long row_fwd_s1(float2 *plane, int ld, const flo
             float e = x[0].x * x[0].x;
 #pragma unroll
             for (int a = 1; a < A; ++a) e = fmaf(x[a].x, x[a].x, e);
-            tt += __float2ll_rn(e * kEnergyScale);
+            tt += __float2ll_rn(fminf(e * scale, kEnergyMax));   // NaN: kEnergyMax
         }
         __syncwarp();
         rdft<A, false>(x);
@@ -447,9 +453,9 @@ __device__ __noinline__ void col_inv_s1(float2 *plane, int ld, const float2 *tw,
 }
 
 // Inverse row pass 1 over the L rows of lags, j fastest, fused with the
-// assembly of Eq. 5: surf holds the window energy's deviation from N^2 (box
-// sums of ||D_sen||^2 - 1) and receives S = (sum T^2 + N^2) - 2 C + deviation;
-// base holds (sum T^2 + N^2) - 2 C's share of frequency 0, as an exact two-part
+// assembly of Eq. 5: surf holds the window energy's deviation from pivot N^2 (box
+// sums of ||D_sen||^2 - pivot) and receives S = (sum T^2 + pivot N^2) - 2 C + deviation;
+// base holds (sum T^2 + pivot N^2) - 2 C's share of frequency 0, as an exact two-part
 // sum, and the product with the (two-part) scale is added to its high part in
 // one rounding.
 template <int NT, int A>
@@ -514,15 +520,119 @@ __device__ __forceinline__ float2 twiddle(int k, int P) {
 
 constexpr int kBoxChunks = 5;   // 160 columns: the usual windows in one go
 
-// Box sums of ||D_sen||^2 - 1 over the N x N template window at every lag
-// (the second term of Eq. 5 less N^2; CFOG vectors have unit norm, so the
-// summands are rounding-sized wherever the image has structure and the sums
-// keep the digits that N^2 would push out).  Rows: a warp takes four rows at a
+// What a 16 x 16 sample of the window and of the template says about their norms.
+// Each of the first eight warps publishes its 32 pixels' largest ||D_sen||^2, how
+// many reach half of that, and their largest T^2, of one channel each; after a
+// barrier every thread reads all eight.  No operation depends on an order or on the
+// CTA's threads.
+constexpr int kSampleSide = 16, kSampleWarps = kSampleSide * kSampleSide / 32;
+struct NormSample {
+    float s[kSampleWarps], t[kSampleWarps];
+    int reach[kSampleWarps];
+};
+__device__ __forceinline__ void sample_norms(const CpView &c, NormSample &o) {
+    const int N = c.N, W = c.N + 2 * c.r;
+    const int i = threadIdx.x / kSampleSide, j = threadIdx.x % kSampleSide;
+    if (i >= kSampleSide) return;
+    const int y = (i * W + W / 2) / kSampleSide, x = (j * W + W / 2) / kSampleSide;
+    const float s = __ldg(c.J.sen_sq + (int64_t)(c.sy0 + y) * c.J.sen_rp + (c.sx0 + x));
+    const float t = __ldg(c.J.ref + (int64_t)(threadIdx.x % c.m) * c.J.ref_pp +
+                    (int64_t)(c.ry0 + (i * N + N / 2) / kSampleSide) * c.J.ref_rp +
+                    (c.rx0 + (j * N + N / 2) / kSampleSide));
+    const float v = fmaxf(s, 0.f), t2 = fmaxf(t * t, 0.f);   // NaN: 0
+    const float s_max = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(v)));
+    const float t_max = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(t2)));
+    const int reach = __popc(__ballot_sync(0xffffffffu, v >= 0.5f * s_max));
+    if ((threadIdx.x & 31) == 0) {
+        o.s[threadIdx.x >> 5] = s_max;
+        o.t[threadIdx.x >> 5] = t_max;
+        o.reach[threadIdx.x >> 5] = reach;
+    }
+}
+
+// Pivot of the box sums: the sample's largest ||D_sen||^2, rounded to eight
+// significant bits, if half of the sample is near it, else 0.  CFOG vectors have
+// the same norm wherever the image has structure (1 unless eps weighs in), so there
+// the summands ||D_sen||^2 - pivot are rounding-sized and the sums keep the digits
+// that pivot N^2 would push out.  Where norms vary a pivot would cost digits
+// instead: with this rule pivot N^2 is a few times the window's energy at most.
+// Eight bits make pivot N^2 an exact float.  Rms error of the box sums, N 128, r 20,
+// of the energies, with pivots of 0, 1 and by this rule (emulated in FP32): unit
+// norm 2e-8, 0, 0; norm 0.03 1.6e-7, 9e-5, 1e-11; 2 % of the window structured
+// 4e-8, 5e-8, 4e-8.  The sample costs 0.5 to 1 % of a CP.
+__device__ __forceinline__ float pivot_of(const NormSample &o) {
+    float top = o.s[0];
+#pragma unroll
+    for (int w = 1; w < kSampleWarps; ++w) top = fmaxf(top, o.s[w]);
+    int n = 0;
+#pragma unroll
+    for (int w = 0; w < kSampleWarps; ++w) n += o.s[w] >= 0.75f * top ? o.reach[w] : 0;
+    const bool use = 2 * n >= kSampleSide * kSampleSide && top > 1e-30f && top < 1e30f;
+    return use ? __uint_as_float((__float_as_uint(top) + 0x8000u) & 0xffff0000u) : 0.f;
+}
+
+// The power of two that brings sum T^2, estimated as N^2 times m times the sample's
+// largest T^2 (N^2 if that is 0), to 2^kEnergyExp or twice that.
+__device__ __forceinline__ float energy_scale(const NormSample &o, int N, int m) {
+    float top = o.t[0];
+#pragma unroll
+    for (int w = 1; w < kSampleWarps; ++w) top = fmaxf(top, o.t[w]);
+    const float est = (top > 0.f ? top * (float)m : 1.f) * ((float)N * (float)N);
+    const int ex = min(max((int)(__float_as_uint(est) >> 23) - 127, kEnergyExp - 120), kEnergyExp + 120);
+    return __uint_as_float((unsigned)(127 + kEnergyExp - ex) << 23);
+}
+
+// sum T^2 in two parts, read from the volume again: 256 partial sums, element e
+// into partial sum e mod 256 of its channel's turn.
+__device__ __noinline__ float2 energy_direct(const CpView &c, float2 *red) {
+    const int tid = threadIdx.x, NN = c.N * c.N;
+    float hi = 0.f, lo = 0.f;
+    for (int k = 0; k < c.m && tid < 256; ++k) {
+        const float *tp = c.J.ref + (int64_t)k * c.J.ref_pp + (int64_t)c.ry0 * c.J.ref_rp + c.rx0;
+        for (int e = tid; e < NN; e += 256) {
+            const float v = __ldg(tp + (int64_t)(e / c.N) * c.J.ref_rp + e % c.N);
+            float err;
+            two_sum(hi, v * v, hi, err);
+            lo += err;
+        }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const float oh = __shfl_xor_sync(0xffffffffu, hi, o), ol = __shfl_xor_sync(0xffffffffu, lo, o);
+        float sum, err;
+        two_sum(hi, oh, sum, err);
+        hi = sum;
+        lo = (lo + ol) + err;
+    }
+    if ((tid & 31) == 0 && tid < 256) red[tid >> 5] = make_float2(hi, lo);
+    __syncthreads();
+    hi = red[0].x;
+    lo = red[0].y;
+    for (int w = 1; w < 8; ++w) {
+        float sum, err;
+        two_sum(hi, red[w].x, sum, err);
+        hi = sum;
+        lo = (lo + red[w].y) + err;
+    }
+    float2 r;
+    two_sum(hi, lo, r.x, r.y);
+    return r;
+}
+
+// Box sums of ||D_sen||^2 - pivot over the N x N template window at every lag
+// (the second term of Eq. 5 less pivot N^2).  Rows: a warp takes four rows at a
 // time, a warp prefix sum each straight from global memory, whose differences
 // at distance N are the row sums.  Columns: up to 256 / L threads per lag
 // column, each sliding over a segment of the row lags.
 template <int NT>
-__device__ __noinline__ void box_sums(const CpView &c, float *scratch, float *out) {
+__device__ __noinline__ void box_sums(CpView &c, NormSample &norms, float *scratch, float *out) {
+    sample_norms(c, norms);
+    __syncthreads();
+    const float pivot = pivot_of(norms);
+    if (threadIdx.x == 0) {
+        c.pivot = pivot;
+        c.scale = energy_scale(norms, c.N, c.m);
+    }
     const int N = c.N, W = N + 2 * c.r, L = 2 * c.r + 1, Lp = L | 1;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     constexpr int NW = NT / 32;
@@ -544,7 +654,7 @@ __device__ __noinline__ void box_sums(const CpView &c, float *scratch, float *ou
 #pragma unroll
                 for (int i = 0; i < kBoxRows; ++i) {
                     const int x = x0 + 32 * ch + lane;
-                    v[i][ch] = x < W ? __ldg(q[i] + x) - 1.f : 0.f;
+                    v[i][ch] = x < W ? __ldg(q[i] + x) - pivot : 0.f;
                 }
 #pragma unroll
             for (int ch = 0; ch < kBoxChunks; ++ch) {
@@ -600,6 +710,28 @@ __device__ __noinline__ void box_sums(const CpView &c, float *scratch, float *ou
     }
 }
 
+// The best kMaxCand of n scores by (value, index), the first of them given: arg-min
+// rounds, each behind the last.  For windows with more lags in the band than the
+// buffer holds (flat or periodic ones), where timing decides which entered it.
+template <int NT>
+__device__ __noinline__ void best_lags(const float *surf, int n, float v0, int i0, float *red_f, int *red_i,
+                                       int *idx) {
+    if (threadIdx.x == 0) idx[0] = i0;
+    for (int c = 1; c < kMaxCand; ++c) {
+        float v = INFINITY;
+        int at = INT_MAX;
+        for (int i = threadIdx.x; i < n; i += NT) {
+            const float sv = surf[i];
+            if ((sv > v0 || (sv == v0 && i > i0)) && (sv < v || (sv == v && i < at))) {
+                v = sv;
+                at = i;
+            }
+        }
+        block_argmin<NT>(v, at, red_f, red_i, v0, i0);
+        if (threadIdx.x == 0) idx[c] = i0;
+    }
+}
+
 // position of frequency f after the forward passes of one axis
 __device__ __forceinline__ int freq_pos(int f, const FftDim &d) { return (f % d.A) * d.B + f / d.A; }
 
@@ -624,8 +756,39 @@ struct CoreShared {
     MatchPlan plan;           // the passes have the register file to themselves
     float dc;                 // accumulated frequency 0 ...
     float dc_err;             // ... and what its sum rounded off
+    float band;               // width of the nomination band
+    float2 base;              // what S has at every lag
+    NormSample norms;
     float zero[kMaxFft];      // a row of zeros
 };
+
+// sum T^2, in two parts, from the threads' integer sums; then the nomination band
+// and, from tid 0, the part of S that is the same at every lag but frequency 0.
+template <class V>
+__device__ __noinline__ void energies(CoreShared<V> &sh, long long part, const float *surf) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    part = warp_sum(part);
+    if (lane == 0) sh.red_l[warp] = part;
+    __syncthreads();
+    long long sum = sh.red_l[0];
+#pragma unroll
+    for (int w = 1; w < V::NT / 32; ++w) sum += sh.red_l[w];
+    const float inv = __uint_as_float((254u << 23) - __float_as_uint(sh.cv.scale));   // 1 / scale
+    const float hi = (float)sum;
+    float2 tt = make_float2(hi * inv, (float)(sum - (long long)hi) * inv);
+    if (sum < kEnergyMin || sum >= (long long)kEnergyMax) tt = energy_direct(sh.cv, &sh.red_cn[0][0]);
+    if (threadIdx.x == 0) {
+        const float N = (float)sh.cv.N, rest = sh.cv.pivot * (N * N);   // exact
+        // the band is relative to the energies that the scores are the difference of:
+        // the template's and the largest of the windows at the corner and middle lags
+        const int L = 2 * sh.cv.r + 1;
+        const float dev = fmaxf(fmaxf(fmaxf(surf[0], surf[L - 1]), fmaxf(surf[L * L - L], surf[L * L - 1])), surf[L * L / 2]);
+        sh.band = kRescoreRel * (tt.x + fmaxf(rest + dev, 0.f));
+        float energy, err;
+        two_sum(tt.x, rest, energy, err);
+        sh.base = make_float2(energy, err + tt.y);
+    }
+}
 
 // The plan of class (N, r, m): the tuned plan when the table holds one and it
 // fits the launch's shared memory; otherwise the cost model's, every thread
@@ -736,7 +899,7 @@ __device__ __forceinline__ void match_one(const MatchArgs &A, const int cp, Core
     float *surf = reinterpret_cast<float *>(twy + Py);   // [Lside^2]
 
     if (tid < min(per_round, DY.nb * DX.nb * m)) sh.item[0][tid] = make_item(cv, plan, tid);
-    box_sums<NT>(cv, planes, surf);
+    box_sums<NT>(sh.cv, sh.norms, planes, surf);
     // twiddles exp(-2 pi i a j / P) at a * B + j: lanes of consecutive j read
     // consecutive values
     const FastDiv divBx(DX.B);
@@ -769,7 +932,7 @@ __device__ __forceinline__ void match_one(const MatchArgs &A, const int cp, Core
                      ((reinterpret_cast<uintptr_t>(J.sen) | reinterpret_cast<uintptr_t>(J.ref)) & 15) == 0;
     const uint32_t tm = sh.tmem + ((uint32_t)(warp & 3) * 32u << 16) +
                         (uint32_t)(warp >> 2) * (uint32_t)(V::COLS / (NT / 128));
-    long long tt_part = 0;   // sum T^2, per thread, fixed point
+    long long tt_part = 0;   // sum T^2, per thread, times sh.scale
     const int items = DY.nb * DX.nb * m;
     const int nrows = DY.bs + 2 * r;
     const int len = raw_len(Px);
@@ -798,11 +961,11 @@ __device__ __forceinline__ void match_one(const MatchArgs &A, const int cp, Core
             float2 *pl = reinterpret_cast<float2 *>(planes + g * pf);
             const int w0 = (warp + g * 3) & (NT / 32 - 1);   // spread the planes' last rows over the warps
 #define CFOG_S1(P_, A_, B_)                                                                         \
-    case P_: tt_part += row_fwd_s1<NT, A_, B_>(pl, ld, twx, divBx, rowD, Py, len, it[g], sh.zero, w0); break;
+    case P_: tt_part += row_fwd_s1<NT, A_, B_>(pl, ld, twx, divBx, rowD, Py, len, it[g], sh.zero, w0, cv.scale); break;
             switch (Px) {
                 CFOG_FFT_LENGTHS(CFOG_S1)
                 default:
-                    CFOG_RADIX_SWITCH(DX.A, (tt_part += row_fwd_s1<NT, RR, 0>(pl, ld, twx, divBx, rowD, Py, len, it[g], sh.zero, w0)));
+                    CFOG_RADIX_SWITCH(DX.A, (tt_part += row_fwd_s1<NT, RR, 0>(pl, ld, twx, divBx, rowD, Py, len, it[g], sh.zero, w0, cv.scale)));
             }
         }
         __syncthreads();
@@ -823,10 +986,9 @@ __device__ __forceinline__ void match_one(const MatchArgs &A, const int cp, Core
         __syncthreads();
     }
 
+    energies<V>(sh, tt_part, surf);
+
     // the inverse passes backwards, then S(v) in surf
-    const auto tt_sum = block_sum<NT>(tt_part, sh.red_l);
-    const float tt_hi = (float)tt_sum;
-    const float tt = tt_hi * (1.0f / kEnergyScale);
     CFOG_RADIX_SWITCH1(DY.B, (col_inv_s2<NT, RR>(plane0, ld, DY.A, divH, sh.cols, tm, &sh.dc)));
     __syncthreads();
     CFOG_RADIX_SWITCH(DY.A, (col_inv_s1<NT, RR>(plane0, ld, twy, DY.B, divP, Lside)));
@@ -842,11 +1004,9 @@ __device__ __forceinline__ void match_one(const MatchArgs &A, const int cp, Core
         scale.x = -0.5f / area;
         scale.y = fmaf(-scale.x, area, -0.5f) / area;
         const float dc = sh.dc, c0 = dc * scale.x;
-        float e1, e2, energy;
-        two_sum(tt, (float)N * (float)N, energy, e1);
-        two_sum(energy, c0, base.x, e2);
-        base.y = e1 + e2 + fmaf(dc, scale.x, -c0) + fmaf(dc, scale.y, sh.dc_err * scale.x) +
-                 (float)(tt_sum - (decltype(tt_sum))tt_hi) * (1.0f / kEnergyScale);
+        float err;
+        two_sum(sh.base.x, c0, base.x, err);
+        base.y = sh.base.y + err + fmaf(dc, scale.x, -c0) + fmaf(dc, scale.y, sh.dc_err * scale.x);
         CFOG_RADIX_SWITCH(DX.A, (row_inv_s1<NT, RR>(plane0, ld, twx, divBx, Lside, scale, base, surf)));
     }
     __syncthreads();
@@ -868,7 +1028,7 @@ __device__ __forceinline__ void match_one(const MatchArgs &A, const int cp, Core
     const bool found = isfinite(smin);
 
     // lags inside the nomination band are re-scored directly
-    const float band = kRescoreRel * (tt + (float)N * (float)N);
+    const float band = sh.band;
     for (int i = tid; i < L2; i += NT) {
         const float sv = surf[i];
         if (found && sv <= smin + band) {
@@ -882,25 +1042,7 @@ __device__ __forceinline__ void match_one(const MatchArgs &A, const int cp, Core
     __syncthreads();
     int ncand = sh.cand_n;
     if (ncand > kCandBuf) {
-        // more lags than the buffer holds (a flat or periodic window), and which of
-        // them entered it depends on timing: the best kMaxCand by (FFT value, index)
-        // are picked from the surface, one arg-min behind the last at a time
-        float pv = smin;
-        int pi = imin;
-        if (tid == 0) sh.cand_idx[0] = imin;
-        for (int c = 1; c < kMaxCand; ++c) {
-            float v = INFINITY;
-            int at = INT_MAX;
-            for (int i = tid; i < L2; i += NT) {
-                const float sv = surf[i];
-                if ((sv > pv || (sv == pv && i > pi)) && (sv < v || (sv == v && i < at))) {
-                    v = sv;
-                    at = i;
-                }
-            }
-            block_argmin<NT>(v, at, sh.red_f, sh.red_i, pv, pi);
-            if (tid == 0) sh.cand_idx[c] = pi;
-        }
+        best_lags<NT>(surf, L2, smin, imin, sh.red_f, sh.red_i, sh.cand_idx);
         ncand = kMaxCand;
     } else if (tid == 0) {
         // order by (FFT value, index) and keep the best kMaxCand
