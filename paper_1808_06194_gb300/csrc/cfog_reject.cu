@@ -3,7 +3,8 @@
 // the residuals and the RMSE, drop the CP with the largest residual, repeat
 // until the RMSE is below the threshold.
 //
-// One CTA of 256 threads per job (1024 when the largest job has 2048 CPs).  The FP64 normal equations are reduced once
+// One CTA per job, of 256 threads or, from 2048 CPs on, of 1024: a job's threads, and
+// with them the order of its sums, depend on its own size only.  The FP64 normal equations are reduced once
 // (warp-cooperative: each lane owns up to three of the 75 sums, the CPs'
 // monomial vectors are staged per warp in shared memory); after that a removal
 // subtracts the dropped CP's terms.  Warp 0 solves by Cholesky in FP64, a row per lane in registers.  The
@@ -25,7 +26,7 @@ namespace cfog {
 namespace {
 
 constexpr int RT = 256;        // threads of a job's CTA ...
-constexpr int RT_BIG = 1024;   // ... and of a launch whose largest job has at least kBigJob CPs
+constexpr int RT_BIG = 1024;   // ... and of a job of at least kBigJob CPs
 constexpr int kBigJob = 2048;
 constexpr int RW = RT / 32;    // warps that reduce the normal equations
 constexpr int kMaxT = 10;                                    // cubic: 10 monomials
@@ -179,15 +180,18 @@ __global__ void __launch_bounds__(NT) reject_kernel(const cfog_point *__restrict
                                                     int min_keep, uint8_t *keep,
                                                     int32_t *__restrict__ order,
                                                     cfog_poly_model *__restrict__ models,
-                                                    float4 *__restrict__ work, int cached) {
+                                                    float4 *__restrict__ work, int cached, int lo, int hi) {
     constexpr int T = PolyDim<DEG>::T;
     constexpr int S = PolyDim<DEG>::S;
     __shared__ RejectShared sh;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int b0 = job_start[blockIdx.x], e0 = job_start[blockIdx.x + 1];
     const int nj = e0 - b0;
+    // a launch for the small jobs may follow: it shares nothing with this one
+    if constexpr (NT == RT_BIG) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    if (nj < lo || nj >= hi) return;   // the other launch's job
     // per-CP state (u, v, first-fit residual), x = NaN for a CP not kept: in
-    // shared memory when the launch reserved room for the largest job
+    // shared memory when the launch reserved room for its largest job
     extern __shared__ float4 wcache[];
     float4 *wb = cached ? wcache : work + b0;
 
@@ -424,6 +428,8 @@ __global__ void __launch_bounds__(NT) reject_kernel(const cfog_point *__restrict
         }
         models[blockIdx.x] = md;
     }
+    // what follows on the stream also follows the big jobs' launch
+    if constexpr (NT != RT_BIG) asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
 size_t offsets_bytes(int32_t n_jobs) { return ((size_t)(n_jobs + 1) * sizeof(int32_t) + 255) / 256 * 256; }
@@ -466,28 +472,54 @@ extern "C" cfog_status cfog_reject_outliers(const cfog_point *cps_dev, const cfo
     cudaStream_t st = as_stream(stream);
     int32_t *off_dev = static_cast<int32_t *>(work_dev);
     float4 *w4 = reinterpret_cast<float4 *>(static_cast<unsigned char *>(work_dev) + offsets_bytes(n_jobs));
-    int32_t max_job = 0;
-    for (int32_t j = 0; j < n_jobs; ++j) max_job = std::max(max_job, job_start[j + 1] - job_start[j]);
-    const size_t cache = (size_t)max_job * sizeof(float4);
-    const int cached = cache <= kCacheMax ? 1 : 0;
-    const int dyn = cached ? (int)cache : 0;
-    // Large jobs take a CTA of 1024 threads: a round's pass over the residuals is
-    // then four times as short (one 10000-CP set, 490 removals: 8.04 ms, before 9.31).
-    const bool big = max_job >= kBigJob;
     using Kernel = void (*)(const cfog_point *, const cfog_match_result *, const int32_t *, double, int, uint8_t *,
-                            int32_t *, cfog_poly_model *, float4 *, int);
+                            int32_t *, cfog_poly_model *, float4 *, int, int, int);
     static const Kernel kernels[2][3] = {
         {reject_kernel<1, RT>, reject_kernel<2, RT>, reject_kernel<3, RT>},
         {reject_kernel<1, RT_BIG>, reject_kernel<2, RT_BIG>, reject_kernel<3, RT_BIG>}};
-    const Kernel kern = kernels[big][degree - 1];
-    const void *fn = reinterpret_cast<const void *>(kern);
-    cfog_status s = ensure_dynamic_smem(fn, dyn, "cfog_reject_outliers");
-    if (s != CFOG_OK) return s;
-    s = check_cuda(cudaMemcpyAsync(off_dev, job_start, (size_t)(n_jobs + 1) * sizeof(int32_t),
+    int32_t max_job[2] = {-1, -1};   // largest job of each launch
+    for (int32_t j = 0; j < n_jobs; ++j) {
+        const int32_t nj = job_start[j + 1] - job_start[j];
+        max_job[nj >= kBigJob] = std::max(max_job[nj >= kBigJob], nj);
+    }
+    size_t cache[2];
+    for (int big = 0; big < 2; ++big) {
+        cache[big] = (size_t)std::max(max_job[big], 0) * sizeof(float4);
+        if (cache[big] > kCacheMax) cache[big] = 0;
+        if (max_job[big] < 0) continue;
+        const cfog_status s = ensure_dynamic_smem(reinterpret_cast<const void *>(kernels[big][degree - 1]),
+                                                  (int)cache[big], "cfog_reject_outliers");
+        if (s != CFOG_OK) return s;
+    }
+    cfog_status s = check_cuda(cudaMemcpyAsync(off_dev, job_start, (size_t)(n_jobs + 1) * sizeof(int32_t),
                                                cudaMemcpyHostToDevice, st),
                                "cfog_reject_outliers: copy of job_start");
     if (s != CFOG_OK) return s;
-    kern<<<n_jobs, big ? RT_BIG : RT, dyn, st>>>(cps_dev, res_dev, off_dev, rmse_threshold, min_keep, keep_dev,
-                                                order_dev, models_dev, w4, cached);
-    return check_launch("cfog_reject_outliers: launch");
+    // Large jobs take a CTA of 1024 threads: a round's pass over the residuals is
+    // then four times as short (one 10000-CP set, 490 removals: 8.04 ms, before 9.31).
+    // Where both kinds occur, the small jobs' launch starts beside the big jobs'
+    // (which leave most of the chip idle) and ends no earlier.
+    for (int big = 1; big >= 0; --big) {
+        if (max_job[big] < 0) continue;
+        cudaLaunchAttribute beside{};
+        beside.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        beside.val.programmaticStreamSerializationAllowed = 1;
+        cudaLaunchConfig_t cfg{};
+        cfg.gridDim = dim3(n_jobs);
+        cfg.blockDim = dim3(big ? RT_BIG : RT);
+        cfg.dynamicSmemBytes = cache[big];
+        cfg.stream = st;
+        cfg.attrs = &beside;
+        cfg.numAttrs = !big && max_job[1] >= 0 ? 1 : 0;
+        s = check_cuda(cudaLaunchKernelEx(&cfg, kernels[big][degree - 1], cps_dev, res_dev,
+                                          (const int32_t *)off_dev, rmse_threshold, (int)min_keep, keep_dev, order_dev,
+                                          models_dev, w4, (int)(max_job[big] == 0 || cache[big] > 0),
+                                          big ? kBigJob : 0, big ? INT_MAX : kBigJob),
+                       "cfog_reject_outliers: launch");
+        if (s != CFOG_OK) {
+            cudaGetLastError();   // a refused launch leaves no error behind
+            return s;
+        }
+    }
+    return CFOG_OK;
 }
