@@ -117,32 +117,53 @@ constexpr int kMinSmem = 77 * 1024;
 constexpr int kTallCps = 2;
 constexpr int kTallSmem = 222 * 1024;   // of the 227 KB a CTA may use, 5 KB for static memory
 
-// Largest dynamic shared memory over every class (N <= tmpl_max, r <=
-// radius_max) of a launch, for the cost-model plan and any tuned plan alike
-// (a device whose table was not written uses the cost model).
-int max_plan_smem(int v, int threads, int tmpl_max, int radius_max, int m) {
-    static std::mutex mu;
-    static std::map<std::array<unsigned, 6>, int> cache;
+// Largest dynamic shared memory over every class (N <= tmpl_max, r <= radius_max)
+// of a launch, for CTAs of kFftThreads and of kFftThreadsTall (-1: a class has no plan).
+struct SmemNeed {
+    int normal, tall;
+    void add(const MatchPlan &p, int N, int r) {
+        normal = std::max(normal, plan_smem_bytes(p, N, r, kFftThreads, p.G));
+        tall = std::max(tall, plan_smem_bytes(p, N, r, kFftThreadsTall, p.G));
+    }
+};
+
+// Over the cost-model plan and any tuned plan alike (a device whose table was not
+// written uses the cost model).  The search over the cost model is made once per
+// bounds; a change of the tuned plans costs a look through the table only.
+SmemNeed max_plan_smem(int v, int tmpl_max, int radius_max, int m) {
+    struct Entry {
+        SmemNeed model, all;
+        unsigned gen;
+    };
+    static std::map<std::array<int, 4>, Entry> cache;   // guarded by the tuning's mutex
     Tuning &T = tuning();
-    std::lock_guard<std::mutex> tl(T.mu);
-    std::lock_guard<std::mutex> lock(mu);
-    const std::array<unsigned, 6> key{(unsigned)v, (unsigned)threads, (unsigned)tmpl_max, (unsigned)radius_max, (unsigned)m, T.gen};
-    auto it = cache.find(key);
-    if (it != cache.end()) return it->second;
+    std::lock_guard<std::mutex> lock(T.mu);
     const PlanLimits lim = variant_limits(v);
-    int best = 0;
-    for (int N = 1; N <= tmpl_max; ++N)
-        for (int r = 0; r <= radius_max; ++r) {
-            MatchPlan p;
-            if (!make_plan_host(N, r, m, lim, &p)) return -1;
-            int b = plan_smem_bytes(p, N, r, threads, p.G);
-            const int e = T.plan[v - 1][N][r];
-            if (e != 0 && (e >> 16) == m && plan_for_code(N, r, m, (e & 0xffff) - 1, lim, &p) >= 0)
-                b = std::max(b, plan_smem_bytes(p, N, r, threads, p.G));
-            best = b > best ? b : best;
-        }
-    cache[key] = best;
-    return best;
+    auto [it, fresh] = cache.try_emplace({v, tmpl_max, radius_max, m}, Entry{{0, 0}, {0, 0}, 0});
+    Entry &e = it->second;
+    if (fresh) {
+        for (int N = 1; N <= tmpl_max && e.model.normal >= 0; ++N)
+            for (int r = 0; r <= radius_max; ++r) {
+                MatchPlan p;
+                if (!make_plan_host(N, r, m, lim, &p)) {
+                    e.model = SmemNeed{-1, -1};
+                    break;
+                }
+                e.model.add(p, N, r);
+            }
+    }
+    if (e.gen != T.gen) {
+        e.gen = T.gen;
+        e.all = e.model;
+        for (int N = 1; N <= tmpl_max && T.count[v - 1] > 0 && e.model.normal >= 0; ++N)
+            for (int r = 0; r <= radius_max; ++r) {
+                MatchPlan p;
+                const int t = T.plan[v - 1][N][r];
+                if (t != 0 && (t >> 16) == m && plan_for_code(N, r, m, (t & 0xffff) - 1, lim, &p) >= 0)
+                    e.all.add(p, N, r);
+            }
+    }
+    return e.all;
 }
 
 // Kernel, shared memory and plan table of a launch of variant v.  One CTA of
@@ -156,11 +177,11 @@ int max_plan_smem(int v, int threads, int tmpl_max, int radius_max, int m) {
 cfog_status prepare(int v, MatchArgs *a, MatchKernel *K) {
     const VariantInfo &info = variant_info(v);
     *K = info.kernel();
-    int smem = max_plan_smem(v, K->threads, a->tmpl_max, a->radius_max, a->m);
+    const SmemNeed need = max_plan_smem(v, a->tmpl_max, a->radius_max, a->m);
+    int smem = need.normal;
     if (info.tall && smem > 0 && (a->n <= kTallCps * sm_count() || smem > variant_limits(v).smem_cap)) {
         *K = info.tall();
-        smem = max_plan_smem(v, K->threads, a->tmpl_max, a->radius_max, a->m);
-        if (smem > 0) smem = std::max(smem, kTallSmem);
+        smem = std::max(need.tall, kTallSmem);
     }
     if (smem <= 0) {
         set_error("cfog_match: no FFT plan for tmpl_max %d radius_max %d", a->tmpl_max, a->radius_max);

@@ -218,9 +218,30 @@ __host__ __device__ inline long long plan_for_code(int N, int r, int m, int code
     return r >= kWideRadius && lim.maxe == kMaxPlaneElems ? cost + cost / 4 : 2 * cost;
 }
 
+// The code of least (cost, code).  A launch searches every class within its bounds
+// once (688k codes for N up to 128 and r up to 20): a code's cost without the charge
+// for its shared memory comes from two short tables, and one that the best so far
+// beats at that is not worked out.
 __host__ inline bool make_plan_host(int N, int r, int m, const PlanLimits &lim, MatchPlan *out) {
+    static_assert(kNbMax == 4 && kPTries == 4, "the digits of a code");
+    const SmoothTable &t = smooth_table();
+    int P[kNbMax][kPTries], len[kNbMax][kPTries];   // lengths of nb blocks (0: none) and their cost
+    for (int n = 0; n < kNbMax; ++n) {
+        const int bs = (N + n) / (n + 1), need = bs + 2 * r;
+        int at = n * bs < N && need <= kMaxFft ? t.next[need] : 0;
+        for (int i = 0; i < kPTries; ++i) {
+            P[n][i] = at;
+            len[n][i] = at ? fft_len_cost(t.A[at], t.B[at]) : 0;
+            at = at ? t.next[at + 1] : 0;
+        }
+    }
     long long best = -1;
     for (int code = 0; code < kPlanCodes; ++code) {
+        const int ny = code >> 4 >> 2, nx = code >> 4 & 3, ty = code >> 2 & 3, tx = code & 3;
+        const int area = P[ny][ty] * P[nx][tx];
+        if (area == 0 || area > lim.maxe) continue;
+        const long long floor_cost = (long long)area * (len[ny][ty] + len[nx][tx]) * ((ny + 1) * (nx + 1) * m + 1);
+        if (best >= 0 && floor_cost >= best) continue;
         MatchPlan p;
         const long long c = plan_for_code(N, r, m, code, lim, &p);
         if (c >= 0 && (best < 0 || c < best)) {
