@@ -172,11 +172,16 @@ __host__ __device__ inline int fft_len_cost(int A, int B) {
 // plan is the code of least cost, ties to the smaller code; the autotuner
 // times codes and records the fastest per class.  A plane that leaves room
 // for one CTA per SM only costs twice as much: it makes every CP of the launch
-// run that way.  Of the 16384-element planes it costs a quarter more from
-// radius kWideRadius on: there a block's window is mostly margin, and small
-// blocks transform up to twice the elements (1000 CPs of N 128, a quarter more
-// against double: r 32 3.0 and 5.3 ms, r 28 2.9 and 3.5, r 24 3.0 and 2.5; 49 CPs:
-// r 28 0.48 and 0.66, r 24 the same).
+// run that way.  Of the 16384-element planes it costs a twelfth more only from
+// radius kWideRadius on: classes of N 57 (r 32: 37) and more have no other plane
+// there but of twice the elements, so a launch with such bounds runs one CTA per SM
+// anyway, and smaller planes mostly transform more for nothing (1000 CPs, a charge of
+// a quarter and of a twelfth: N 78, r 26 1.67 and 1.58 ms, N 76, r 27 1.76 and 1.58,
+// N 176, r 26 5.65 and 5.18; N 99, r 26, whose small planes are 7 % dearer, 2.31 with
+// them and 2.34 without; the double charge: N 128, r 32 5.3 ms, now 3.0).  Below it the
+// double charge pays (1000 CPs of N 128, r 24: 2.5 ms, without 3.0), though not for few
+// CPs, whose launches run one CTA per SM in any case (49 of N 72, r 23: 0.20 ms, with
+// the larger plane 0.155): a CP's plan does not depend on its launch.
 constexpr int kWideRadius = 26;
 constexpr int kPlanCodes = kNbMax * kNbMax * kPTries * kPTries;
 
@@ -215,7 +220,7 @@ __host__ __device__ inline long long plan_for_code(int N, int r, int m, int code
     const long long per = (long long)Py * Px * (fft_len_cost(Ay, By) + fft_len_cost(Ax, Bx));
     const long long cost = per * (long long)(items + 1);
     if (fixed <= lim.smem_cap) return cost;
-    return r >= kWideRadius && lim.maxe == kMaxPlaneElems ? cost + cost / 4 : 2 * cost;
+    return r >= kWideRadius && lim.maxe == kMaxPlaneElems ? cost + cost / 12 : 2 * cost;
 }
 
 // The code of least (cost, code).  A launch searches every class within its bounds
