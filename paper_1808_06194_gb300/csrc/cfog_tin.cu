@@ -344,10 +344,12 @@ __device__ __forceinline__ bool tile_outside(int px, int py, int qx, int qy, int
 __global__ void tin_setup_kernel(const cfog_point *__restrict__ cps, const cfog_match_result *__restrict__ res,
                                  const int32_t *__restrict__ tris, int n_tris, int n_cps, int out_h,
                                  int out_w, TinWork wk) {
-    const int t = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
-    if (t >= n_tris) return;
+    const unsigned u = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    if (u >= (unsigned)n_tris) return;
+    const int t = (int)u, lane = threadIdx.x & 31;
     TinTri T{};
-    const int ia = tris[3 * t], ib = tris[3 * t + 1], ic = tris[3 * t + 2];
+    const int32_t *v = tris + 3 * (size_t)t;
+    const int ia = v[0], ib = v[1], ic = v[2];
     T.ok = 0;
     if (ia < 0 || ib < 0 || ic < 0 || ia >= n_cps || ib >= n_cps || ic >= n_cps) {
         if (lane == 0) wk.tri[t] = T;
