@@ -39,11 +39,13 @@ RMIN, RMAX = 8, 20
 MARGIN = 64 + RMAX + 16   # half template + radius + largest true offset
 SEED_PAIR = 1
 SEED_CP = 101
-# DRAM read + write bytes per CP of the batched matcher, from an ncu capture of
-# 1024 CPs of this workload (dram__bytes_read.sum + dram__bytes_write.sum =
-# 1125.34 MB + 17.23 MB).  Set to None when the kernel changes.
-MATCH_TRAFFIC_PER_CP = 1142.57e6 / 1024
-MATCH_TRAFFIC_NOTE = "DRAM bytes of one ncu capture of a 1024-CP launch (1142.6 MB), scaled by CP count"
+# DRAM read + write bytes per CP of the batched matcher (wide variant with tuned
+# plans, the autotuner's pick on GB300), from an ncu capture of 1024 CPs of this
+# workload (dram__bytes_read.sum + dram__bytes_write.sum = 1052.28 MB + 17.06 MB).
+# Set to None when the kernel changes.
+MATCH_TRAFFIC_PER_CP = 1069.34e6 / 1024
+MATCH_TRAFFIC_NOTE = ("DRAM bytes of one ncu capture of a 1024-CP launch (1069.3 MB, wide variant with tuned "
+                      "plans), scaled by CP count")
 E2E_PIPE_STEPS = 40   # timed steps per pipelined end-to-end run (three runs, median)
 WORKLOAD = "batched 2048x2048 f32 pair, 1024 Harris CPs (32x32 grid), N in {48,64,96,128}, r in 8..20"
 

@@ -63,8 +63,8 @@ enum {
     CFOG_CP_EDGE_PEAK = 2,   /* minimum on the border of the search window:
                                 integer offset kept, no sub-pixel refinement    */
     CFOG_CP_FLAT = 3,        /* reserved                                        */
-    CFOG_CP_TIMEOUT = 4,     /* a bounded device-side wait gave up: the result is
-                                not valid                                       */
+    CFOG_CP_TIMEOUT = 4,     /* a bounded wait of the tensor-core path gave up:
+                                the result is not valid                         */
     CFOG_CP_NONFINITE = 5    /* no lag has a finite score (NaN or infinite pixels in
                                 the template or window): no match, the prior kept,
                                 ssd infinite                                    */
@@ -114,6 +114,8 @@ typedef struct {
  *   sqnorm     ||D(y,x)||^2 at sqnorm[y*row_pitch + x] (written by
  *              cfog_extract, read by cfog_match)
  *   row_pitch  in floats, a multiple of 4; plane_pitch in floats, >= h*row_pitch
+ * cfog_extract writes vectors of norm 1 (0 where nothing varies, less where eps
+ * weighs in).  cfog_match takes finite vectors of any norm, with their own sqnorm.
  * cfog_feature_layout() gives the layout cfog_extract expects.                 */
 typedef struct {
     float *data;

@@ -11,10 +11,13 @@
 // block-wide arg-max then pick the chip's k best (ties: smaller y, then
 // smaller x).  Every sum runs over its taps in ascending order.
 //
-// What bounds it: FP32 arithmetic, 54 FMA per pixel of the two filters, plus
-// about 20 other instructions.  Nothing but the image row crosses memory; the
-// tiled form before it read every filter tap from shared memory (60 loads per
-// pixel, 33 % of the issue slots arithmetic).  8192^2 u16 pixels, 41 x 41
+// What bounds it: the issue slots (65 % used at 8192^2, 16 warps per SM) and the
+// image rows' latency (2.1 of 5.8 stall cycles per issue).  145 thread instructions
+// per pixel, 54 of them the FMA of the two filters; strips of 56 columns over a
+// 197-column cell and eight extra rows per segment add 1.3 and 1.1 times.  The FMA
+// pipe is 39 % busy, DRAM at 5 % of the copy rate: nothing but the image row crosses
+// memory.  The tiled form before it read every filter tap from shared memory (60
+// loads per pixel, 33 % of the issue slots arithmetic).  8192^2 u16 pixels, 41 x 41
 // cells: 1.20 -> 0.40 ms; 2048^2 f32, 32 x 32 cells: 67 -> 42 us; the same with
 // eight points a cell 1.48 -> 0.67 ms and 97 -> 91 us.
 #include "cfog_internal.cuh"

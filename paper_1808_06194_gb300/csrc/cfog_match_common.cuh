@@ -1,4 +1,4 @@
-// Device code shared by the FFT matcher (cfog_match.cu) and the BF16
+// Device code shared by the FFT matcher (cfog_match_fft.cuh) and the BF16
 // tensor-core matcher (cfog_bf16.cu): launch arguments, job views, block
 // reductions, the sub-pixel fit.  Internal to libcfog.
 #pragma once
