@@ -185,13 +185,13 @@ __device__ __forceinline__ void stage_items(const Item *items, int64_t srp, int6
     X(144, 12, 12) X(160, 16, 10) X(180, 15, 12)
 
 // sum T^2 is a sum of integers, which does not depend on which thread took which
-// row: lanes' shares of a row times a power of two that brings the CP's sum, as a
-// sample of the template estimates it, to 2^38 or twice that.  From 2^32 on the
-// shares' rounding is below a float's, and up to 2^20 shares of at most 2^42 add
-// up.  A sum outside [2^32, 2^42) (the sample saw a part of the template that is
-// far from the rest) is taken again by energy_direct.
-constexpr int kEnergyExp = 38;
-constexpr long long kEnergyMin = 1LL << 32;
+// row: lanes' shares of a row times a power of two that brings N^2 m times the largest
+// T^2 of a sample to 2^40 or twice that (CFOG sums reach an eighth of it).  From 2^28 on
+// the shares' rounding is below a float's, unless a few pixels that the sample took
+// for typical outshine the rest (1e-7 then), and up to 2^20 shares of at most 2^42
+// add up.  A sum outside [2^28, 2^42) is taken again by energy_direct.
+constexpr int kEnergyExp = 40;
+constexpr long long kEnergyMin = 1LL << 28;
 constexpr float kEnergyMax = 4398046511104.f;      // 2^42
 
 // Row pass 1 (radix A at stride B) on one plane, reading the raw pixels in
@@ -520,81 +520,58 @@ __device__ __forceinline__ float2 twiddle(int k, int P) {
 
 constexpr int kBoxChunks = 5;   // 160 columns: the usual windows in one go
 
-// What a 16 x 16 sample of the window and of the template says about their norms.
-// Each of the first eight warps publishes its 32 pixels' largest ||D_sen||^2, how
-// many reach half of that, and their largest T^2, of one channel each; after a
-// barrier every thread reads all eight.  No operation depends on an order or on the
-// CTA's threads.
-constexpr int kSampleSide = 16, kSampleWarps = kSampleSide * kSampleSide / 32;
-struct NormSample {
-    float s[kSampleWarps], t[kSampleWarps];
-    int reach[kSampleWarps];
-};
-__device__ __forceinline__ void sample_norms(const CpView &c, NormSample &o) {
+// Pivot of the box sums and scale of sum T^2, from a sample of 32 pixels of the
+// window and of the template, one per lane (a row and a column each).  Every warp
+// takes the same sample: no barrier, and nothing depends on the CTA's threads.
+//
+// Pivot: the sample's largest ||D_sen||^2, rounded to eight significant bits, if
+// three quarters of the sample reach half of it, else 0.  CFOG vectors have the same
+// norm wherever the image has structure (1 unless eps weighs in), so there the
+// summands ||D_sen||^2 - pivot are rounding-sized and the sums keep the digits that
+// pivot N^2 would push out.  Where norms vary a pivot costs digits instead.  Eight
+// bits make pivot N^2 an exact float.  Rms error of the box sums, N 128, r 20, of the
+// energies, with pivots of 0, 1 and by the rule (emulated in FP32): unit norm 2e-8, 0,
+// 0; norm 0.03 1.6e-7, 9e-5, 1e-11; 40 % of the window flat 7e-9, 4e-8, 7e-9; 98 % flat
+// 4e-8, 5e-8, 4e-8.
+//
+// Scale: the power of two that brings N^2 times m times the sample's largest T^2, of
+// a channel per lane (N^2 if that is 0), to 2^kEnergyExp or twice that.
+__device__ __forceinline__ float2 sample_norms(const CpView &c) {
+    const int lane = threadIdx.x & 31, col = (13 * lane + 5) & 31;
     const int N = c.N, W = c.N + 2 * c.r;
-    const int i = threadIdx.x / kSampleSide, j = threadIdx.x % kSampleSide;
-    if (i >= kSampleSide) return;
-    const int y = (i * W + W / 2) / kSampleSide, x = (j * W + W / 2) / kSampleSide;
-    const float s = __ldg(c.J.sen_sq + (int64_t)(c.sy0 + y) * c.J.sen_rp + (c.sx0 + x));
-    const float t = __ldg(c.J.ref + (int64_t)(threadIdx.x % c.m) * c.J.ref_pp +
-                    (int64_t)(c.ry0 + (i * N + N / 2) / kSampleSide) * c.J.ref_rp +
-                    (c.rx0 + (j * N + N / 2) / kSampleSide));
+    const float s = __ldg(c.J.sen_sq + (int64_t)(c.sy0 + (lane * W + W / 2) / 32) * c.J.sen_rp +
+                          (c.sx0 + (col * W + W / 2) / 32));
+    const float t = __ldg(c.J.ref + (int64_t)(lane % c.m) * c.J.ref_pp +
+                          (int64_t)(c.ry0 + (lane * N + N / 2) / 32) * c.J.ref_rp + (c.rx0 + (col * N + N / 2) / 32));
     const float v = fmaxf(s, 0.f), t2 = fmaxf(t * t, 0.f);   // NaN: 0
-    const float s_max = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(v)));
-    const float t_max = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(t2)));
-    const int reach = __popc(__ballot_sync(0xffffffffu, v >= 0.5f * s_max));
-    if ((threadIdx.x & 31) == 0) {
-        o.s[threadIdx.x >> 5] = s_max;
-        o.t[threadIdx.x >> 5] = t_max;
-        o.reach[threadIdx.x >> 5] = reach;
-    }
-}
-
-// Pivot of the box sums: the sample's largest ||D_sen||^2, rounded to eight
-// significant bits, if half of the sample is near it, else 0.  CFOG vectors have
-// the same norm wherever the image has structure (1 unless eps weighs in), so there
-// the summands ||D_sen||^2 - pivot are rounding-sized and the sums keep the digits
-// that pivot N^2 would push out.  Where norms vary a pivot would cost digits
-// instead: with this rule pivot N^2 is a few times the window's energy at most.
-// Eight bits make pivot N^2 an exact float.  Rms error of the box sums, N 128, r 20,
-// of the energies, with pivots of 0, 1 and by this rule (emulated in FP32): unit
-// norm 2e-8, 0, 0; norm 0.03 1.6e-7, 9e-5, 1e-11; 2 % of the window structured
-// 4e-8, 5e-8, 4e-8.  The sample costs 0.5 to 1 % of a CP.
-__device__ __forceinline__ float pivot_of(const NormSample &o) {
-    float top = o.s[0];
-#pragma unroll
-    for (int w = 1; w < kSampleWarps; ++w) top = fmaxf(top, o.s[w]);
-    int n = 0;
-#pragma unroll
-    for (int w = 0; w < kSampleWarps; ++w) n += o.s[w] >= 0.75f * top ? o.reach[w] : 0;
-    const bool use = 2 * n >= kSampleSide * kSampleSide && top > 1e-30f && top < 1e30f;
-    return use ? __uint_as_float((__float_as_uint(top) + 0x8000u) & 0xffff0000u) : 0.f;
-}
-
-// The power of two that brings sum T^2, estimated as N^2 times m times the sample's
-// largest T^2 (N^2 if that is 0), to 2^kEnergyExp or twice that.
-__device__ __forceinline__ float energy_scale(const NormSample &o, int N, int m) {
-    float top = o.t[0];
-#pragma unroll
-    for (int w = 1; w < kSampleWarps; ++w) top = fmaxf(top, o.t[w]);
-    const float est = (top > 0.f ? top * (float)m : 1.f) * ((float)N * (float)N);
+    const float top = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(v)));
+    const float t_top = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(t2)));
+    const bool use = __popc(__ballot_sync(0xffffffffu, v >= 0.5f * top)) >= 24 && top > 1e-30f && top < 1e30f;
+    const float est = (t_top > 0.f ? t_top * (float)c.m : 1.f) * ((float)N * (float)N);
     const int ex = min(max((int)(__float_as_uint(est) >> 23) - 127, kEnergyExp - 120), kEnergyExp + 120);
-    return __uint_as_float((unsigned)(127 + kEnergyExp - ex) << 23);
+    return make_float2(use ? __uint_as_float((__float_as_uint(top) + 0x8000u) & 0xffff0000u) : 0.f,
+                       __uint_as_float((unsigned)(127 + kEnergyExp - ex) << 23));
 }
 
-// sum T^2 in two parts, read from the volume again: 256 partial sums, element e
-// into partial sum e mod 256 of its channel's turn.
+// sum T^2 in two parts, read from the volume again.  Eight warps take the rows of
+// every channel in turn, four rows' loads at a time.
 __device__ __noinline__ float2 energy_direct(const CpView &c, float2 *red) {
-    const int tid = threadIdx.x, NN = c.N * c.N;
+    const int tid = threadIdx.x, lane = tid & 31, N = c.N;
     float hi = 0.f, lo = 0.f;
     for (int k = 0; k < c.m && tid < 256; ++k) {
         const float *tp = c.J.ref + (int64_t)k * c.J.ref_pp + (int64_t)c.ry0 * c.J.ref_rp + c.rx0;
-        for (int e = tid; e < NN; e += 256) {
-            const float v = __ldg(tp + (int64_t)(e / c.N) * c.J.ref_rp + e % c.N);
-            float err;
-            two_sum(hi, v * v, hi, err);
-            lo += err;
-        }
+        for (int y = tid >> 5; y < N; y += 32)
+            for (int x = lane; x < N; x += 32) {
+                float v[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) v[u] = y + 8 * u < N ? __ldg(tp + (int64_t)(y + 8 * u) * c.J.ref_rp + x) : 0.f;
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    float err;
+                    two_sum(hi, v[u] * v[u], hi, err);
+                    lo += err;
+                }
+            }
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
@@ -625,13 +602,12 @@ __device__ __noinline__ float2 energy_direct(const CpView &c, float2 *red) {
 // at distance N are the row sums.  Columns: up to 256 / L threads per lag
 // column, each sliding over a segment of the row lags.
 template <int NT>
-__device__ __noinline__ void box_sums(CpView &c, NormSample &norms, float *scratch, float *out) {
-    sample_norms(c, norms);
-    __syncthreads();
-    const float pivot = pivot_of(norms);
+__device__ __noinline__ void box_sums(CpView &c, float *scratch, float *out) {
+    const float2 norms = sample_norms(c);
+    const float pivot = norms.x;
     if (threadIdx.x == 0) {
         c.pivot = pivot;
-        c.scale = energy_scale(norms, c.N, c.m);
+        c.scale = norms.y;
     }
     const int N = c.N, W = N + 2 * c.r, L = 2 * c.r + 1, Lp = L | 1;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -758,7 +734,6 @@ struct CoreShared {
     float dc_err;             // ... and what its sum rounded off
     float band;               // width of the nomination band
     float2 base;              // what S has at every lag
-    NormSample norms;
     float zero[kMaxFft];      // a row of zeros
 };
 
@@ -899,7 +874,7 @@ __device__ __forceinline__ void match_one(const MatchArgs &A, const int cp, Core
     float *surf = reinterpret_cast<float *>(twy + Py);   // [Lside^2]
 
     if (tid < min(per_round, DY.nb * DX.nb * m)) sh.item[0][tid] = make_item(cv, plan, tid);
-    box_sums<NT>(sh.cv, sh.norms, planes, surf);
+    box_sums<NT>(sh.cv, planes, surf);
     // twiddles exp(-2 pi i a j / P) at a * B + j: lanes of consecutive j read
     // consecutive values
     const FastDiv divBx(DX.B);

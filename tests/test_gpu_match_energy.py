@@ -96,15 +96,16 @@ def test_windows_constant_but_for_a_patch():
     _check(torch, P, fa, fb, np.array([(128, 130), (120, 122)], np.int32), 160, 16)
 
 
-@pytest.mark.parametrize("at,gain", [((20, 21), 1e5), ((20, 21), 100.0), ((22, 22), 1e5), ((22, 22), 200.0)])
+@pytest.mark.parametrize("at,gain", [((20, 21), 1e5), ((20, 21), 100.0), ((22, 22), 1e5), ((22, 22), 200.0),
+                                     ((21, 15), 1e5), ((21, 15), 200.0)])
 def test_template_energy_in_a_few_pixels(at, gain):
-    """Energy that a 4-pixel sampling of the 64 x 64 template misses (rows and columns 4 i, 4 i + 1)
-    or takes for typical (a single pixel at 4 i + 2)."""
+    """Energy that a sample of the 64 x 64 template misses (even rows) or takes for
+    typical (a sampled pixel, row 21 and column 15)."""
     torch, P = cuda_or_skip()
     oracle.build()
     fa, fb = (P.cfog_extract(to_dev(torch, im)) for im in _images())
     fa = _scaled(fa, 1.0)
-    k = 1 if at[0] % 4 == 2 else 2
+    k = 2 if at == (20, 21) else 1
     y, x = PTS[0, 1] - 32 + at[0], PTS[0, 0] - 32 + at[1]
     fa.volume()[:, y:y + k, x:x + k] *= gain
     _check(torch, P, fa, fb, PTS[:1], 64, 12)
