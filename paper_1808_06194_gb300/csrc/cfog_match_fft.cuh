@@ -907,7 +907,7 @@ __device__ __forceinline__ void match_one(const MatchArgs &A, const int cp, Core
                      ((reinterpret_cast<uintptr_t>(J.sen) | reinterpret_cast<uintptr_t>(J.ref)) & 15) == 0;
     const uint32_t tm = sh.tmem + ((uint32_t)(warp & 3) * 32u << 16) +
                         (uint32_t)(warp >> 2) * (uint32_t)(V::COLS / (NT / 128));
-    long long tt_part = 0;   // sum T^2, per thread, times sh.scale
+    long long tt_part = 0;   // sum T^2, per thread, times cv.scale
     const int items = DY.nb * DX.nb * m;
     const int nrows = DY.bs + 2 * r;
     const int len = raw_len(Px);
